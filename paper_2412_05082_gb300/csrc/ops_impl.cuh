@@ -76,10 +76,11 @@ static inline void fx_host_row(const double* c, int n, double factor, int f, int
   for (int t = 0; t < n; ++t) out[t] = fx_host(v[t], 0, kFxBand);
 }
 
-// smallest e with v < 2^e
+// smallest e with v < 2^e, v a little enlarged: a coefficient's high limb has to
+// stay below 2^31
 static inline int fx_ceil_exp(double v) {
   int e;
-  std::frexp(v, &e);
+  std::frexp(v * (1.0 + 1e-8), &e);
   return e;
 }
 
@@ -176,7 +177,7 @@ static bool make_fx(HostTables<double, K>* h, const std::vector<double>& dinv, i
       h->fx->Sf[j][c] = fwd(0, j, c);
       h->fx->Sb[j][c] = bwd(0, j, c);
     }
-  h->fx->eax = -2 - s.gy;
+  h->fx->eax = -s.gy;
   h->fx->corr = std::pow(s.cf * s.cb, d);
   full->canon = *h->fx;
   // sweeps: every row at its own scale
@@ -207,7 +208,7 @@ static bool make_fx(HostTables<double, K>* h, const std::vector<double>& dinv, i
         full->Sf[ty][j][c] = fwd(ty, j, c);
         full->Sb[ty][j][c] = bwd(ty, j, c);
       }
-  full->eax = -2 - s.gy;
+  full->eax = -s.gy;
   full->corr = std::pow(s.cf * s.cb, d);
   std::vector<double> ds(md);  // the division, with the column scales taken back
   for (int slot = 0; d == 2 && slot < slots; ++slot) {
