@@ -182,6 +182,7 @@ static bool make_fx(HostTables<double, K>* h, const std::vector<double>& dinv, i
   full->canon = *h->fx;
   // sweeps: every row at its own scale
   int2* bx[3] = {h->band.M, h->band.L, h->band.B};
+  float* ba[3] = {h->band.aM, h->band.aL, h->band.aB};
   for (int o = 0; o < 3; ++o)
     for (int c = 0; c < NC; ++c) {
       double sum = 0.0;
@@ -191,8 +192,11 @@ static bool make_fx(HostTables<double, K>* h, const std::vector<double>& dinv, i
       fx_host_row(tab[o][c], BW, 1.0, f, full->s[o][c]);
       if (c >= K) continue;
       h->band.f[o][c] = f;
-      for (int t = band_lo(o, c, K); t <= band_hi(o, c, K); ++t)
+      for (int t = band_lo(o, c, K); t <= band_hi(o, c, K); ++t) {
         bx[o][FxIdx<K>::at(o, c, t)] = full->s[o][c][t + 2 * K];
+        ba[o][FxIdx<K>::at(o, c, t)] =
+            (float)std::ldexp(std::fabs(tab[o][c][t + 2 * K]), f - kFxCoef);
+      }
     }
   full->band = h->band;
   // every class and type

@@ -78,6 +78,50 @@ def apply(d, mats, x):
     return y
 
 
+def graded(kind, shape, at, rng):
+    """Uniform values times a field that changes by many powers of two."""
+    x = rng.uniform(-1, 1, shape)
+    n = shape[-1]
+    if kind == "spike":
+        x[tuple(min(at, m - 1) for m in shape)] = 2.0 ** 70
+    elif kind == "jump":
+        x[..., at:] *= 2.0 ** 30
+    elif kind == "jump_last":
+        x[at:] *= 2.0 ** 30
+    else:
+        x *= 2.0 ** np.linspace(-80, 80, n)
+    return x
+
+
+# the spike and the jumps at every cell of a block of four cells
+@pytest.mark.parametrize("d,k,L", [(2, 3, 4), (2, 4, 3), (2, 7, 3), (3, 3, 3), (3, 5, 2)])
+@pytest.mark.parametrize("kind", ["spike", "jump", "jump_last", "ramp"])
+def test_operator_rows_are_accurate_to_their_own_values(bh, d, k, L, kind):
+    """Every row of A x and of b - A x within n u sum |a_ij| |x_j|, n the roundings
+    of a chain of FP64 sums, wherever larger values lie on the line."""
+    N = 2 ** L
+    n = k * N - 1
+    mats = line_matrices(bh, k, N)
+    absm = [np.abs(m) for m in mats]
+    rng = np.random.default_rng(10 * k + d)
+    tol = (d * (4 * k + 2) + 6) * U
+    with bh.Context(bh.default_params(d, k, L)) as ctx:
+        for cell in range(0, 4 if kind != "ramp" else 1):
+            x = graded(kind, (n,) * d, k * cell + cell % k, rng)
+            X, Y = cuda(x), torch.empty(n ** d, dtype=torch.float64, device="cuda")
+            ctx.apply_A(L, X, Y)
+            scale = float(N) ** (4 - d)
+            y = Y.cpu().numpy().reshape(x.shape)
+            ref = apply(d, mats, x.astype(LD)) * LD(scale)
+            size = (apply(d, absm, np.abs(x)) * scale)
+            assert (np.abs((y - ref).astype(np.float64)) <= tol * size).all(), cell
+            b = np.ldexp(rng.uniform(-1, 1, x.shape), np.frexp(size)[1])
+            ctx.residual(L, X, cuda(b), Y)
+            r = Y.cpu().numpy().reshape(x.shape)
+            err = np.abs((r - (b.astype(LD) - ref)).astype(np.float64))
+            assert (err <= tol * (size + np.abs(b))).all(), cell
+
+
 def color0_patches(k, N):
     """(x slice, y slice, vertex) of the patches of color 0."""
     m = 2 * k - 1
