@@ -159,3 +159,31 @@ def test_step_at_a_smooth_solution_moves_it_no_further_than_fp64(bh, k, tile):
         moved += (got[sy, sx] ** 2).sum()
         fp64 += (np.linalg.solve(A, r64[sy, sx].ravel()) ** 2).sum()
     assert moved <= fp64, (np.sqrt(moved), np.sqrt(fp64))
+
+
+@pytest.mark.parametrize("tile", [0, 5])
+@pytest.mark.parametrize("k", [2, 4, 7])
+@pytest.mark.parametrize("kind", ["spike", "jump", "jump_last", "ramp"])
+def test_step_at_a_graded_solution_is_accurate_patch_by_patch(bh, k, kind, tile):
+    """One color at solutions that change by 2^30 and more over a few nodes: every
+    patch moves by less than FP64's bound for its own residual (n u sum |a_ij| |x_j|)
+    carried through the inverse of the patch."""
+    L, N = 4, 16
+    n = k * N - 1
+    mats = line_matrices(bh, k, N)
+    absm = [np.abs(m) for m in mats]
+    rng = np.random.default_rng(k)
+    tol = (2 * (4 * k + 2) + 6 + 4 * (2 * k - 1)) * U
+    with bh.Context(bh.default_params(2, k, L)) as ctx:
+        ctx.set_tile(tile)
+        for at in (k * 8 - 1, k * 8 + k // 2, k * 9 - 1):
+            x = graded(kind, (n, n), at, rng)
+            b = apply(2, mats, x.astype(LD)).astype(np.float64)
+            size = apply(2, absm, np.abs(x))
+            X = cuda(x)
+            ctx.smooth_colors(L, X, cuda(b * float(N) ** 2), 0, 1)
+            got = np.abs(X.cpu().numpy().reshape(n, n) - x)
+            for sx, sy in color0_patches(k, N):
+                inv = np.abs(np.linalg.inv(local_matrix(mats, sx, sy)))
+                bound = tol * (inv @ size[sy, sx].ravel()) + U * np.abs(x[sy, sx]).ravel()
+                assert (got[sy, sx].ravel() <= bound).all(), (at, sx.start, sy.start)
