@@ -116,7 +116,8 @@ __global__ void __launch_bounds__(256) mvs2_batch_kernel(Meta m, const MvsArgs<T
     if (!m.active[p]) continue;
     const auto* tb = static_cast<const Tables<T, K>*>(m.tabs[p]);
     if constexpr (sizeof(T) == 8) {
-      fx2_any_tile<K>(bc.c, tb, args[tl.s], tl.first, tl.count, smem_raw);
+      fx2_any_tile<K>(bc.c, tb, args[tl.s], tl.first, tl.count,
+                      args[tl.s].count <= kFx2SmallCount, smem_raw);
     } else if (mvs2_tile_is_interior(args[tl.s], tl.first, tl.count)) {
       mvs2_tile_interior<T, K, true>(bc.c, bc.c, args[tl.s], tl.first, tl.count, smem_raw);
     } else {
@@ -399,7 +400,8 @@ __global__ void __launch_bounds__(256, 2) vcycle_persistent_kernel(
     const auto* tb = static_cast<const Tables<T, KK>*>(mT.tabs[p]);                           \
     if constexpr (sizeof(T) == 8)                                                             \
       fx2_any_tile<KK>(static_cast<const FxFull<KK>*>(args[tile.s].fx)->canon, tb,            \
-                       args[tile.s], tile.first, tile.count, smem_raw);                       \
+                       args[tile.s], tile.first, tile.count,                                  \
+                       args[tile.s].count <= kFx2SmallCount, smem_raw);                       \
     else if (KK <= kBatchInteriorMaxK && mvs2_tile_is_interior(args[tile.s], tile.first, tile.count)) \
       mvs2_tile_interior<T, KK>(tb->op, tb->fdm, args[tile.s], tile.first, tile.count, smem_raw); \
     else                                                                                      \

@@ -155,3 +155,33 @@ def test_operator_scales_exactly_and_spreads_nan(bh, d, k, L):
         got = torch.isnan(residual(x, b)).cpu().numpy()
         assert np.all(got[(A[:, n // 2].toarray().ravel() != 0)])
         assert got.sum() <= (4 * k + 1) ** d
+
+
+@pytest.mark.parametrize("k,tile", [(2, 32), (3, 9), (4, 17), (5, 5), (6, 9), (7, 8)])
+def test_requested_tile_takes_the_throughput_form(bh, k, tile):
+    """A tile that is asked for is computed by the throughput form on any level, so
+    that small problems reach it: its scales and folded lines round differently from
+    the latency form that a level with few patches takes by itself, to the same
+    result; and it hands patches over to the FP64 form."""
+    L = 4
+    n1 = k * 2 ** L - 1
+    n = n1 * n1
+    A = assemble.c0ip_matrix(2, k, 2 ** L)
+    loc = LocalSolvers(assemble.c0ip_matrix(2, k, 2 ** L, mixed=False), 2, k, 2 ** L)
+    x, b = workload.vector_uniform(n, 21), workload.rhs_uniform(n, 22)
+    ref = smoothers.mvs_step(A, loc, b, x, 1.0)
+    small = smooth(bh, 2, k, L, cuda(x), cuda(b), 0)
+    got = smooth(bh, 2, k, L, cuda(x), cuda(b), tile)
+    assert not torch.equal(got, small)
+    for v in (got, small):
+        assert np.abs(v.cpu().numpy() - ref).max() <= 1e-10 * np.abs(ref - x).max()
+    # one value out of range: the patches around it in FP64, the others of their tiles
+    # unchanged (the middle of the domain, all patches there away from the boundary)
+    far = x.copy()
+    far[n // 2] = 2.0 ** 800
+    hit = smooth(bh, 2, k, L, cuda(far), cuda(b), tile).cpu().numpy()
+    assert np.isfinite(hit).all()
+    assert np.array_equal(hit[:k], got.cpu().numpy()[:k])
+    far[n // 2] = np.nan
+    hit = smooth(bh, 2, k, L, cuda(far), cuda(b), tile).cpu().numpy()
+    assert np.isnan(hit[n // 2]) and np.isfinite(hit[:k]).all()
