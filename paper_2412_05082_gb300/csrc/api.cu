@@ -137,8 +137,7 @@ template <typename T>
 bh_status patches_t(bh_ctx* c, int l, const T* r, T* x, int lo, int hi, bool atomic) {
   Level& L = c->lv[l];
   const double sc = c->p.omega * L.pscale;
-  if (c->p.local_solver == BH_EXACT && c->exact_gemm &&
-      (sizeof(T) == 8 || c->coarse_n >= kExactGemmMinF32)) {
+  if (c->p.local_solver == BH_EXACT && c->exact_gemm) {
     // per color in [lo, hi): gather the patch tensors as columns, Y = sc Ainv R
     // (dense products by runs of one type combination, gemm.cu), scatter-add Y
     const int md = c->coarse_n;  // (2k - 1)^d, the size of every patch

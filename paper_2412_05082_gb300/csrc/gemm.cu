@@ -5,7 +5,7 @@
 //
 //   Y = alpha * A R,   A: m^d x m^d symmetric;  R, Y: m^d x cnt, column-major,
 //
-// with m^d from 49 (2D k = 4) to 2197 (3D k = 7).
+// with m^d = 729, 1331, 2197 for 3D k = 5, 6, 7.
 //
 // FP64: emulated on the FP16 tensor cores by splitting the operands into
 // integer slices (an error-free splitting of the Ozaki type).  Every row of A

@@ -187,3 +187,23 @@ def test_step_at_a_graded_solution_is_accurate_patch_by_patch(bh, k, kind, tile)
                 inv = np.abs(np.linalg.inv(local_matrix(mats, sx, sy)))
                 bound = tol * (inv @ size[sy, sx].ravel()) + U * np.abs(x[sy, sx]).ravel()
                 assert (got[sy, sx].ravel() <= bound).all(), (at, sx.start, sy.start)
+
+
+@pytest.mark.parametrize("d,k", [(2, 4), (2, 7), (3, 3), (3, 4)])
+def test_exact_solver_keeps_every_entry_of_its_inverse(bh, d, k):
+    """On the single patch of level 1 the correction of a unit vector is a column of
+    the patch inverse, a symmetric matrix: entry (i, j) from column j and entry (j, i)
+    from column i agree to rounding, however much smaller than the largest entry of
+    its row it is."""
+    n = (2 * k - 1) ** d
+    Y = np.empty((n, n))
+    with bh.Context(bh.default_params(d, k, 1, local_solver=bh.EXACT)) as ctx:
+        x = torch.empty(n, dtype=torch.float64, device="cuda")
+        b = torch.zeros(n, dtype=torch.float64, device="cuda")
+        for j in range(n):
+            x.zero_()
+            b.zero_()
+            b[j] = 1.0
+            ctx.smooth(1, x, b, 1)
+            Y[j] = x.cpu().numpy()
+    assert (np.abs(Y - Y.T) <= 4 * U * np.abs(Y)).all()
