@@ -93,8 +93,12 @@ struct FxScales {
   double cf, cb;  // largest absolute sums of the forward and backward eigenvector lines
 };
 
-// exponent e_c of the forward lines' column scale 2^-e_c (about l_c^(-1/2))
-static inline int fx_col_exp(double lam) { return (int)std::lround(0.5 * std::log2(lam)); }
+// exponent e_c of the forward lines' column scale 2^-e_c (about l_c^(-1/2)).  The
+// eigenvalues are 20 and more with the default penalty; with a small one they may
+// be negative or near zero.
+static inline int fx_col_exp(double lam) {
+  return (int)std::lround(0.5 * std::log2(std::max(std::fabs(lam), 1.0)));
+}
 
 template <int K>
 static FxScales fx_scales(const OpTab<double, K>& op, const FdmTab<double, K>& fdm, int classes,
@@ -221,7 +225,7 @@ static bool make_fx(HostTables<double, K>* h, const std::vector<double>& dinv, i
       int e = 0, ll = l, ss = slot;
       for (int a = 0; a < d; ++a, ll /= M, ss /= 4) e += fx_col_exp(fdm.lam[ss % 4][ll % M]);
       ds[l] = std::ldexp(dinv[(size_t)slot * md + l], e);
-      top = std::max(top, ds[l]);
+      top = std::max(top, std::fabs(ds[l]));
     }
     full->cD[slot] = top * (1.0 + 1e-9);
     const long double inv = 1.0L / full->cD[slot];

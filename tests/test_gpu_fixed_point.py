@@ -185,3 +185,23 @@ def test_requested_tile_takes_the_throughput_form(bh, k, tile):
     far[n // 2] = np.nan
     hit = smooth(bh, 2, k, L, cuda(far), cuda(b), tile).cpu().numpy()
     assert np.isnan(hit[n // 2]) and np.isfinite(hit[:k]).all()
+
+
+@pytest.mark.parametrize("k,gamma", [(2, 1.0), (2, 1.04), (2, 1.2), (2, 60.0), (3, 5.0), (4, 500.0)])
+@pytest.mark.parametrize("tile", [0, 6])
+def test_penalties_that_leave_negative_eigenvalues(bh, k, gamma, tile):
+    """A penalty below the default can leave the 1D patch matrices at the boundary
+    indefinite (negative eigenvalues at Q2 with 1.0 to 1.2) while the coarse matrix
+    is positive definite; larger ones widen the spectrum."""
+    L = 3
+    n = (k * 2 ** L - 1) ** 2
+    A = assemble.c0ip_matrix(2, k, 2 ** L, gamma)
+    loc = LocalSolvers(assemble.c0ip_matrix(2, k, 2 ** L, gamma, mixed=False), 2, k, 2 ** L)
+    x, b = workload.vector_uniform(n, 31), workload.rhs_uniform(n, 32)
+    ref = smoothers.mvs_step(A, loc, b, x, 1.0)
+    with bh.Context(bh.default_params(2, k, L, gamma=gamma)) as ctx:
+        ctx.set_tile(tile)
+        X = cuda(x)
+        ctx.smooth(L, X, cuda(b), 1)
+        got = X.cpu().numpy()
+    assert np.abs(got - ref).max() <= 1e-10 * np.abs(ref - x).max()
