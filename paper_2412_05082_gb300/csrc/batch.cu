@@ -507,15 +507,19 @@ size_t mvs_smem(int k, int pb, bool persistent = false) {
   }
 }
 
+// the patch kernel's configuration: FP64 in fixed point, FP32 on its own pipe
+template <typename T, int K>
+using MvsCfg = std::conditional_t<sizeof(T) == 8, Fx2Cfg<K>, Mvs2Cfg<T, K>>;
+
 template <typename T>
 int mvs_pb_max_t(int k) {
   switch (k) {
-    case 2: return Mvs2Cfg<T, 2>::PB_MAX;
-    case 3: return Mvs2Cfg<T, 3>::PB_MAX;
-    case 4: return Mvs2Cfg<T, 4>::PB_MAX;
-    case 5: return Mvs2Cfg<T, 5>::PB_MAX;
-    case 6: return Mvs2Cfg<T, 6>::PB_MAX;
-    default: return Mvs2Cfg<T, 7>::PB_MAX;
+    case 2: return MvsCfg<T, 2>::PB_MAX;
+    case 3: return MvsCfg<T, 3>::PB_MAX;
+    case 4: return MvsCfg<T, 4>::PB_MAX;
+    case 5: return MvsCfg<T, 5>::PB_MAX;
+    case 6: return MvsCfg<T, 6>::PB_MAX;
+    default: return MvsCfg<T, 7>::PB_MAX;
   }
 }
 

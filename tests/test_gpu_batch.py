@@ -436,3 +436,24 @@ def test_batched_solve_does_not_read_basis_vectors_it_never_formed(bh):
         with bh.Batch(params) as batch:
             _, rrs = batch.solve(bs, xs, 1e-8, 100)
             assert all(r <= 1.0001e-8 for r in rrs), rrs
+
+
+@pytest.mark.parametrize("k,most", [(2, 32), (4, 27), (5, 17), (6, 12), (7, 8)])
+def test_largest_tile_of_the_batch_is_that_of_its_kernel(bh, k, most):
+    """The FP64 patch kernel of a batch holds `most` patches of degree k in 110 KB
+    of shared memory; that tile is accepted, one more is refused, and the V-cycle of a
+    level whose colors exceed 1,024 patches (the throughput form) equals that of the
+    smallest tile (a result does not depend on the tile)."""
+    L = 7
+    n = (k * 2 ** L - 1) ** 2
+    b = cuda(workload.rhs_uniform(n, 900 + k))
+    x1, x2 = torch.empty_like(b), torch.empty_like(b)
+    with bh.Batch([bh.default_params(2, k, L)]) as batch:
+        batch.set_tile(k, most)
+        if most < 32:
+            with pytest.raises(bh.BiharmError):
+                batch.set_tile(k, most + 1)
+        batch.vcycle([b], [x1])
+        batch.set_tile(k, 1)
+        batch.vcycle([b], [x2])
+        assert relerr(host(x1), host(x2)) <= 1e-12
