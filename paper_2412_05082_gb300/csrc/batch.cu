@@ -166,8 +166,10 @@ struct MvsOp {
   DevArray<MvsArgs<T>> args;
   DevArray<int> pid;
   DevArray<Tile> tiles;
-  size_t smem = 0;            // shared memory of a launch, and of the persistent kernel's tiles
-  size_t psmem = 0;
+  DevArray<MvsArgs<T>> pargs;  // FP64: those of the persistent kernel
+  DevArray<Tile> ptiles;
+  size_t smem = 0;            // shared memory of a launch
+  size_t psmem = 0;           // and of the persistent kernel's tiles
   int k = 0;                  // the degree of every problem of the op
   const void* htab = nullptr;  // their common interior tables (host copy; the kernel parameter)
 };
@@ -487,29 +489,21 @@ int mvs_pb(const bh_batch* b, int k) {
   return b->mixed ? 4 : kFx2Tile[k];  // default before tuning
 }
 
-// shared memory of the graph form's patch kernel (FP64: the fixed-point form,
-// Fx2Cfg) and of the persistent kernel's tiles
-template <typename T, int K>
-size_t mvs_smem_k(int pb, bool persistent) {
-  const size_t fx = Fx2Cfg<K>::smem_bytes(pb), fl = Mvs2Cfg<T, K>::smem_bytes(pb);
-  return sizeof(T) == 4 ? fl : (persistent ? std::max(fx, fl) : fx);
-}
-
-template <typename T>
-size_t mvs_smem(int k, int pb, bool persistent = false) {
-  switch (k) {
-    case 2: return mvs_smem_k<T, 2>(pb, persistent);
-    case 3: return mvs_smem_k<T, 3>(pb, persistent);
-    case 4: return mvs_smem_k<T, 4>(pb, persistent);
-    case 5: return mvs_smem_k<T, 5>(pb, persistent);
-    case 6: return mvs_smem_k<T, 6>(pb, persistent);
-    default: return mvs_smem_k<T, 7>(pb, persistent);
-  }
-}
-
 // the patch kernel's configuration: FP64 in fixed point, FP32 on its own pipe
 template <typename T, int K>
 using MvsCfg = std::conditional_t<sizeof(T) == 8, Fx2Cfg<K>, Mvs2Cfg<T, K>>;
+
+template <typename T>
+size_t mvs_smem(int k, int pb) {
+  switch (k) {
+    case 2: return MvsCfg<T, 2>::smem_bytes(pb);
+    case 3: return MvsCfg<T, 3>::smem_bytes(pb);
+    case 4: return MvsCfg<T, 4>::smem_bytes(pb);
+    case 5: return MvsCfg<T, 5>::smem_bytes(pb);
+    case 6: return MvsCfg<T, 6>::smem_bytes(pb);
+    default: return MvsCfg<T, 7>::smem_bytes(pb);
+  }
+}
 
 template <typename T>
 int mvs_pb_max_t(int k) {
@@ -558,9 +552,9 @@ bh_status build_vdepth(bh_batch* b, int t, VDepth<T>& V, Depth& D) {
   // agree byte for byte, i.e. of one penalty): patch-list arguments, problems,
   // tiles
   struct Group {
-    std::vector<MvsArgs<T>> args;
+    std::vector<MvsArgs<T>> args, pargs;
     std::vector<int> pid;
-    std::vector<Tile> tiles;
+    std::vector<Tile> tiles, ptiles;
     const void* htab = nullptr;
   };
   std::map<std::tuple<int, int, int>, Group> groups;  // (color, degree, table class)
@@ -584,7 +578,7 @@ bh_status build_vdepth(bh_batch* b, int t, VDepth<T>& V, Depth& D) {
     const int k = b->k[p];
     const int pb = std::min(mvs_pb(b, k), mvs_pb_max_t<T>(k));
     smem_k[k] = mvs_smem<T>(k, pb);
-    psmem_k[k] = mvs_smem<T>(k, pb, true);
+    psmem_k[k] = mvs_smem<T>(k, sizeof(T) == 8 ? std::min(pb, kPersistentTile) : pb);
     const DevTables dt = Ops<T>::device_tables(LvBuf<T>::tab(c), k);
     // one launch per class of problems whose interior tables agree byte for
     // byte (one penalty), the tables being the launch's parameter
@@ -618,6 +612,12 @@ bh_status build_vdepth(bh_batch* b, int t, VDepth<T>& V, Depth& D) {
       const int step = sizeof(T) == 8 && a.count <= kFx2SmallCount ? 1 : pb;
       for (int f = (a.count - 1) / step * step; a.count > 0 && f >= 0; f -= step)
         G.tiles.push_back(Tile{s, f, std::min(step, a.count - f)});
+      if (sizeof(T) == 8) {
+        a.pb = std::min(pb, kPersistentTile);
+        G.pargs.push_back(a);
+        for (int f = 0, pt = std::min(step, kPersistentTile); f < a.count; f += pt)
+          G.ptiles.push_back(Tile{s, f, std::min(pt, a.count - f)});
+      }
     }
   }
   if (!p0.empty()) {
@@ -632,6 +632,10 @@ bh_status build_vdepth(bh_batch* b, int t, VDepth<T>& V, Depth& D) {
       BCKS(upload(b, G.args, op.args));
       BCKS(upload(b, G.pid, op.pid));
       BCKS(upload(b, G.tiles, op.tiles));
+      if (sizeof(T) == 8) {
+        BCKS(upload(b, G.pargs, op.pargs));
+        BCKS(upload(b, G.ptiles, op.ptiles));
+      }
       op.smem = smem_k[k];
       op.psmem = psmem_k[k];
       op.k = k;
@@ -1066,11 +1070,12 @@ struct PhaseBuilder {
         P.kind = kPhMvs;
       }
       MvsGroup& G = P.groups[P.ngroups++];
-      G.args = op.args.d;
+      G.args = sizeof(T) == 8 ? op.pargs.d : op.args.d;
       G.pid = op.pid.d;
-      G.tiles = op.tiles.d;
-      G.ntiles = op.tiles.n;
-      P.total += op.tiles.n;
+      const DevArray<Tile>& tiles = sizeof(T) == 8 ? op.ptiles : op.tiles;
+      G.tiles = tiles.d;
+      G.ntiles = tiles.n;
+      P.total += tiles.n;
       smem = std::max(smem, op.psmem);
     }
     ph.push_back(P);
@@ -1128,7 +1133,7 @@ bh_status build_phases(bh_batch* b, const TopOps& top) {
   BCKS(upload(b, ph, dph));
   b->d_phases = dph.d;
   b->nphases = (int)ph.size();
-  b->psmem = std::max<size_t>(B.smem, 8 * FxSweepCfg<kMaxK, 2>::VALUES);
+  b->psmem = std::max<size_t>(B.smem, sizeof(T) == 8 ? 8 * FxSweepCfg<kMaxK, 2>::VALUES : 64);
   // co-resident grid of the cooperative launch; the kernel's shared-memory
   // limit is only ever raised (other live batches may launch it with more)
   const void* kernel = vcycle_persistent_kernel_for<T>();

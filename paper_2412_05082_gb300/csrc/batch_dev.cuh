@@ -300,6 +300,36 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned* gen, uns
   return ok != 0;
 }
 
+// Patches per tile of the persistent kernel in FP64 at most (1, 2, 4: 93, 72, 61 ms
+// for a V-cycle of 64 problems; 8: 92, its shared memory leaves one block per SM).
+constexpr int kPersistentTile = 4;
+
+// thread `t` of a 32-line x 4-cell tile (block blk) of a 2D sweep, with plain loads:
+// the inputs were written by an earlier phase
+template <int K, int KIND>
+__device__ __forceinline__ void sweep_tile_coherent(const OpTab<double, K>& op,
+                                                    const SweepArgs<double>& a, int64_t blk,
+                                                    int t) {
+  const int tc = (a.N + kSplitTileCells - 1) / kSplitTileCells;
+  const int64_t lt = blk / tc, l = lt * kSplitTileLines + t % kSplitTileLines;
+  const int c = (int)(blk - lt * tc) * kSplitTileCells + t / kSplitTileLines;
+  if (l >= a.lines || c >= a.N) return;
+  const int64_t base = a.axis == 0 ? l * a.n : l;
+  if (c >= 2 && c <= a.N - 2) {
+    sweep_cell<double, K, KIND, true, true>(op, a, base, c, nullptr);
+  } else {
+    int cls[K];
+#pragma unroll
+    for (int q = 0; q < K; ++q) cls[q] = c * K + q >= 1 ? row_class<K>(c * K + q, a.N) : 0;
+    sweep_cell<double, K, KIND, false, true>(op, a, base, c, cls);
+  }
+}
+
+// One kernel holds the code of every degree (128 registers, spills), so the tiles
+// take the form of the fixed-point smoother with the least of it, the latency form,
+// and the defects of the FP32 V-cycle the FP64 sweeps.  A V-cycle of 64 problems: FP64
+// with the graph's unrolled tiles 74 ms, on the FP64 pipe 68, this way 61 (the graph
+// 38); FP32 with FP64 defects 27 with fixed-point sweeps, 24 this way.
 template <typename T>
 __global__ void __launch_bounds__(256, 2) vcycle_persistent_kernel(
     Meta m64, Meta mT, const Phase* __restrict__ phases, int nphases, unsigned* bar,
@@ -312,22 +342,32 @@ __global__ void __launch_bounds__(256, 2) vcycle_persistent_kernel(
     const int kind = P.kind;
     if (kind == kPhSweep0 || kind == kPhSweep2) {
       const SweepArgs<double>* args = static_cast<const SweepArgs<double>*>(P.args);
-      for (int64_t q = blockIdx.x; q < P.total / kSplitBlock; q += gridDim.x) {
+      // FP64: a block's first 128 threads take a fixed-point tile, as the graph; the
+      // FP32 V-cycle's defects: two 128-thread tiles on the FP64 pipe
+      const int per = sizeof(T) == 8 ? 1 : 2;
+      for (int64_t q = per * blockIdx.x + (per - 1) * (threadIdx.x / kSplitBlock);
+           q < P.total / kSplitBlock; q += per * gridDim.x) {
         const int s = find_seg(P.prefix, P.n, q * kSplitBlock);
         const int p = P.pid[s];
         if (!m64.active[p]) continue;
         const int64_t blk = q - P.prefix[s] / kSplitBlock;
-        const SweepArgs<double> a = args[s];
-        double* sh = reinterpret_cast<double*>(smem_raw);
-        __syncthreads();  // the previous block's values are still read
+        if (sizeof(T) == 8) __syncthreads();  // the previous tile's values are still read
 #define BH_CALL(KK)                                                                          \
   {                                                                                          \
-    const auto& full = *static_cast<const FxFull<KK>*>(a.fx);                                \
     const auto* op = &static_cast<const Tables<double, KK>*>(m64.tabs[p])->op;               \
-    if (kind == kPhSweep0)                                                                   \
-      fxs_block<KK, 0, true>(full.band, full, op, a, blk, sh);                               \
-    else                                                                                     \
-      fxs_block<KK, 2, true>(full.band, full, op, a, blk, sh);                               \
+    if constexpr (sizeof(T) == 8) {                                                          \
+      const SweepArgs<double> a = args[s];                                                   \
+      const auto& full = *static_cast<const FxFull<KK>*>(a.fx);                              \
+      double* sh = reinterpret_cast<double*>(smem_raw);                                      \
+      if (kind == kPhSweep0)                                                                 \
+        fxs_block<KK, 0, true>(full.band, full, op, a, blk, sh);                             \
+      else                                                                                   \
+        fxs_block<KK, 2, true>(full.band, full, op, a, blk, sh);                             \
+    } else if (kind == kPhSweep0) {                                                          \
+      sweep_tile_coherent<KK, 0>(*op, args[s], blk, threadIdx.x % kSplitBlock);              \
+    } else {                                                                                 \
+      sweep_tile_coherent<KK, 2>(*op, args[s], blk, threadIdx.x % kSplitBlock);              \
+    }                                                                                        \
   }
         BH_KSWITCH(m64.k[p], BH_CALL)
 #undef BH_CALL
@@ -399,9 +439,7 @@ __global__ void __launch_bounds__(256, 2) vcycle_persistent_kernel(
   {                                                                                           \
     const auto* tb = static_cast<const Tables<T, KK>*>(mT.tabs[p]);                           \
     if constexpr (sizeof(T) == 8)                                                             \
-      fx2_any_tile<KK>(static_cast<const FxFull<KK>*>(args[tile.s].fx)->canon, tb,            \
-                       args[tile.s], tile.first, tile.count,                                  \
-                       args[tile.s].count <= kFx2SmallCount, smem_raw);                       \
+      fx2_small_tile<KK>(tb, args[tile.s], tile.first, tile.count, smem_raw);                 \
     else if (KK <= kBatchInteriorMaxK && mvs2_tile_is_interior(args[tile.s], tile.first, tile.count)) \
       mvs2_tile_interior<T, KK>(tb->op, tb->fdm, args[tile.s], tile.first, tile.count, smem_raw); \
     else                                                                                      \

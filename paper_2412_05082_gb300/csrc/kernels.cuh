@@ -230,7 +230,7 @@ __device__ __forceinline__ void sweep_cell(const OpTab<T, K>& tab, const SweepAr
 }
 
 // one thread of a sweep: thread index tid in [0, lines * N)
-template <typename T, int K, int KIND, bool COHERENT = false>
+template <typename T, int K, int KIND>
 __device__ __forceinline__ void sweep_thread(const OpTab<T, K>& tab, const SweepArgs<T>& a,
                                              int64_t tid) {
   int64_t line;
@@ -246,7 +246,7 @@ __device__ __forceinline__ void sweep_thread(const OpTab<T, K>& tab, const Sweep
   int64_t strides[3] = {1, (int64_t)a.n, (int64_t)a.n * a.n};
   const int64_t base = line_offset(line, a.d, a.axis, dims, strides);
   if (c >= 2 && c <= a.N - 2) {
-    sweep_cell<T, K, KIND, true, COHERENT>(tab, a, base, c, nullptr);
+    sweep_cell<T, K, KIND, true>(tab, a, base, c, nullptr);
   } else {
     int cls[K];
 #pragma unroll
@@ -254,7 +254,7 @@ __device__ __forceinline__ void sweep_thread(const OpTab<T, K>& tab, const Sweep
       const int g = c * K + q;
       cls[q] = (g >= 1) ? row_class<K>(g, a.N) : 0;
     }
-    sweep_cell<T, K, KIND, false, COHERENT>(tab, a, base, c, cls);
+    sweep_cell<T, K, KIND, false>(tab, a, base, c, cls);
   }
 }
 

@@ -457,3 +457,36 @@ def test_largest_tile_of_the_batch_is_that_of_its_kernel(bh, k, most):
         batch.set_tile(k, 1)
         batch.vcycle([b], [x2])
         assert relerr(host(x1), host(x2)) <= 1e-12
+
+
+@pytest.mark.parametrize("persistent", [False, True])
+def test_batched_forms_outside_the_fixed_point_range(bh, persistent):
+    """Right-hand sides beyond the exponents of the fixed-point kernels take the FP64
+    form of their sweeps and tiles in the graph's kernels (2^720), a spike of 2^80 that
+    of single patches and cells; a NaN stays in its own problem."""
+    probs = [(2, 2, 7), (2, 3, 3), (2, 5, 2), (2, 7, 3)]
+    bs = [workload.rhs_uniform((k * 2 ** L - 1) ** 2, 950 + i) for i, (d, k, L) in enumerate(probs)]
+    with bh.Batch([bh.default_params(d, k, L) for d, k, L in probs]) as batch:
+        batch.set_persistent(persistent)
+
+        def vcycle(vs):
+            X = [torch.empty_like(v) for v in vs]
+            batch.vcycle(vs, X)
+            return [host(x) for x in X]
+
+        ref = vcycle([cuda(b) for b in bs])
+        for got, r in zip(vcycle([cuda(b) * 2.0 ** 720 for b in bs]), ref):
+            assert relerr(got * 2.0 ** -720, r) <= 1e-10
+        spiked = [b.copy() for b in bs]
+        for b in spiked:
+            b[len(b) // 2] = 2.0 ** 80
+        # linear: the spike alone plus the rest, to FP64's rounding of the spike
+        alone = [np.where(np.arange(len(b)) == len(b) // 2, b, 0.0) for b in spiked]
+        for got, r in zip(vcycle([cuda(b) for b in spiked]), vcycle([cuda(b) for b in alone])):
+            assert relerr(got, r) <= 1e-10
+        B = [cuda(b) for b in bs]
+        B[1][0] = float("nan")
+        got = vcycle(B)
+        assert np.isnan(got[1]).any()
+        for i in (0, 2, 3):
+            assert np.array_equal(got[i], ref[i])
