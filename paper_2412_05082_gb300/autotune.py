@@ -13,14 +13,24 @@ concurrently and compete for the SMs, so the best tile of a degree can depend
 on the mix.
 
 Results are cached as JSON keyed by dimension, degree (or the batch's
-problem list) and device architecture, in $BIHARM_TUNE_CACHE or
-~/.cache/biharm_gb300/tiles.json.
+problem list), device architecture and the library's device code, in
+$BIHARM_TUNE_CACHE or ~/.cache/biharm_gb300/tiles.json.
 """
 
+import functools
+import glob
+import hashlib
 import json
+import math
 import os
 
-CANDIDATES = (1, 2, 3, 4, 6, 8, 12, 16, 24, 32)
+# with the tiles at which one FP64 smoothing step of each degree is fastest (9, 11,
+# 17, 25; kFx2Tile in mvs_fx.cuh) among them
+CANDIDATES = (1, 2, 3, 4, 6, 8, 9, 11, 12, 16, 17, 24, 25, 32)
+
+# kFx2SmallCount (mvs_fx.cuh): colors of up to this many patches are computed one
+# patch per block in FP64, whatever the tile
+SMALL_COLOR = 1024
 
 
 def cache_path():
@@ -30,10 +40,23 @@ def cache_path():
     return os.path.join(os.path.expanduser("~"), ".cache", "biharm_gb300", "tiles.json")
 
 
+@functools.lru_cache(maxsize=1)
+def _kernels():
+    """A digest of the library's sources: tiles tuned for other kernels are not taken
+    over."""
+    h = hashlib.sha1()
+    for path in sorted(glob.glob(os.path.join(os.path.dirname(os.path.abspath(__file__)),
+                                              "csrc", "*"))):
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:12]
+
+
 def _arch():
     import torch
     cap = torch.cuda.get_device_capability()
-    return "sm_%d%d_%s" % (cap[0], cap[1], torch.cuda.get_device_name().replace(" ", "_"))
+    return "sm_%d%d_%s_%s" % (cap[0], cap[1], torch.cuda.get_device_name().replace(" ", "_"),
+                              _kernels())
 
 
 def load_cache():
@@ -59,7 +82,10 @@ def tune_degree(k, level=None, problems=4, reps=5, verbose=False, precision=0):
     import torch
     import paper_2412_05082_gb300 as bh
     if level is None:  # about 2e5 unknowns per problem
-        level = max(2, min(9, int(round(__import__("math").log2(450.0 / k)))))
+        level = max(2, min(9, int(round(math.log2(450.0 / k)))))
+        # a level whose colors (an eighth of the patches) depend on the tile
+        while precision == 0 and (2 ** level - 1) ** 2 // 8 <= SMALL_COLOR:
+            level += 1
     params = [bh.default_params(2, k, level, precision=precision) for _ in range(problems)]
     times = {}
     with bh.Batch(params) as batch:

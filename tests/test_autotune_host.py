@@ -81,3 +81,49 @@ def test_unreadable_cache_is_treated_as_empty(tuner):
     batch = FakeBatch(best={2: 3}, limit={})
     assert autotune.tune_batch(batch, [(2, 2, 4)]) == {2: 3}
     assert json.load(open(tuner))  # rewritten as valid JSON
+
+
+class FakeDegreeBatch(FakeBatch):
+    """The batch that tune_degree builds, with the level it was built for."""
+    levels = []
+
+    def __init__(self, params):
+        super().__init__(best={p.degree: 8 for p in params}, limit={})
+        FakeDegreeBatch.levels.append(params[0].level)
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *exc):
+        pass
+
+
+@pytest.mark.parametrize("k", range(2, 8))
+def test_a_degree_is_tuned_where_its_tile_matters(tuner, monkeypatch, k):
+    """In FP64 the colors of the tuned level exceed 1,024 patches: below, the library
+    takes one patch per block whatever the tile."""
+    import torch
+    monkeypatch.setattr(bh, "Batch", FakeDegreeBatch)
+    monkeypatch.setattr(torch.cuda, "synchronize", lambda: None)
+    best, times = autotune.tune_degree(k)
+    assert best == 8 and sorted(times) == sorted(autotune.CANDIDATES)
+    patches = (2 ** FakeDegreeBatch.levels[-1] - 1) ** 2
+    assert patches // 8 > 1024
+
+
+def test_cached_tiles_belong_to_the_kernels_they_were_tuned_for(monkeypatch, tmp_path):
+    import torch
+    monkeypatch.setattr(torch.cuda, "get_device_capability", lambda: (10, 3))
+    monkeypatch.setattr(torch.cuda, "get_device_name", lambda: "Fake GB300")
+    here = autotune._arch()
+    assert here.startswith("sm_103_Fake_GB300")
+    (tmp_path / "csrc").mkdir()
+    (tmp_path / "csrc" / "other.cuh").write_text("// other kernels")
+    monkeypatch.setattr(autotune, "__file__", str(tmp_path / "autotune.py"))
+    autotune._kernels.cache_clear()
+    assert autotune._arch() != here
+    autotune._kernels.cache_clear()
+
+
+def test_the_default_tiles_are_candidates():
+    assert {32, 25, 17, 11, 9, 8} <= set(autotune.CANDIDATES)
