@@ -728,7 +728,6 @@ bh_status bh_create(const bh_params* params, void* stream, bh_ctx** out) {
     L.g.n = k * L.g.N - 1;
     L.g.nd = ipow64(L.g.n, d);
     L.ascale = std::pow((double)L.g.N, 4 - d);
-    L.fx = Ops<double>::device_tables(c->tab64, k).fx;
     L.pscale = 1.0 / L.ascale;
     const size_t nd = (size_t)L.g.nd;
     if ((status = dmalloc(c, &L.x64, nd)) || (status = dmalloc(c, &L.b64, nd)) ||

@@ -247,6 +247,7 @@ struct bh_batch {
   // device meta
   int* d_k = nullptr;
   const void** d_tabs64 = nullptr;
+  const void** d_fx = nullptr;
   const void** d_tabs32 = nullptr;
   const void** d_tabsff = nullptr;  // RC: FfTab<k> per problem
   int* d_active = nullptr;
@@ -297,7 +298,7 @@ bh_status upload(bh_batch* b, const std::vector<A>& h, DevArray<A>& d) {
 
 template <typename T>
 Meta meta(const bh_batch* b) {
-  return Meta{b->d_k, sizeof(T) == 8 ? b->d_tabs64 : b->d_tabs32, b->d_active};
+  return Meta{b->d_k, sizeof(T) == 8 ? b->d_tabs64 : b->d_tabs32, b->d_fx, b->d_active};
 }
 
 unsigned blocks_for(int64_t threads, int bs) { return (unsigned)((threads + bs - 1) / bs); }
@@ -335,7 +336,6 @@ SweepArgs<T> sweep_args(const Level& Lv, int axis, const T* in0, const T* in1, c
   a.stride = axis == 0 ? 1 : Lv.g.n;
   a.axis = axis;
   a.scale = Lv.ascale;
-  a.fx = Lv.fx;
   a.mode = mode;
   a.b = bvec;
   a.in[0] = in0;
@@ -1397,21 +1397,24 @@ bh_status bh_batch_create(const bh_params* params, int count, void* stream, bh_b
     b->k.push_back(p.degree);
     b->L.push_back(p.level);
   }
-  std::vector<const void*> tabs64, tabs32, tabsff;
+  std::vector<const void*> tabs64, tabsfx, tabs32, tabsff;
   for (int p = 0; p < count; ++p) {
-    tabs64.push_back(Ops<double>::device_tables(b->ctx[p]->tab64, b->k[p]).tables);
+    const DevTables dt = Ops<double>::device_tables(b->ctx[p]->tab64, b->k[p]);
+    tabs64.push_back(dt.tables);
+    tabsfx.push_back(dt.fx);
     tabs32.push_back(b->mixed ? Ops<float>::device_tables(b->ctx[p]->tab32, b->k[p]).tables
                               : nullptr);
     tabsff.push_back(b->rc ? ff_device_tables(b->ctx[p]->tab32, b->k[p]) : nullptr);
   }
   DevArray<int> dk;
-  DevArray<const void*> dt64, dt32, dtff;
+  DevArray<const void*> dt64, dtfx, dt32, dtff;
   bh_status s;
-  if ((s = upload(b, b->k, dk)) || (s = upload(b, tabs64, dt64)) || (s = upload(b, tabs32, dt32)) ||
-      (s = upload(b, tabsff, dtff)))
+  if ((s = upload(b, b->k, dk)) || (s = upload(b, tabs64, dt64)) || (s = upload(b, tabsfx, dtfx)) ||
+      (s = upload(b, tabs32, dt32)) || (s = upload(b, tabsff, dtff)))
     return bail(s);
   b->d_k = dk.d;
   b->d_tabs64 = dt64.d;
+  b->d_fx = dtfx.d;
   b->d_tabs32 = dt32.d;
   b->d_tabsff = dtff.d;
   std::vector<int> act(count, 1);

@@ -19,6 +19,7 @@ namespace bdev {
 struct Meta {                 // per problem, indexed by problem id
   const int* k;               // degree
   const void* const* tabs;    // Tables<T, K>* (device) of the launch's value type
+  const void* const* fx;      // FxFull<K>* (device), the fixed-point tables of FP64 launches
   const int* active;          // 0: problem finished, skip it
 };
 
@@ -49,7 +50,7 @@ __global__ void __launch_bounds__(128, 4) sweep_batch_kernel(Meta m, const Sweep
   const SweepArgs<double> a = args[s];
 #define BH_CALL(KK)                                                                       \
   {                                                                                       \
-    const auto& full = *static_cast<const FxFull<KK>*>(a.fx);                             \
+    const auto& full = *static_cast<const FxFull<KK>*>(m.fx[p]);                          \
     fxs_block<KK, KIND>(full.band, full, &static_cast<const Tables<double, KK>*>(m.tabs[p])->op, \
                         a, blk, sh);                                                      \
   }
@@ -357,7 +358,7 @@ __global__ void __launch_bounds__(256, 2) vcycle_persistent_kernel(
     const auto* op = &static_cast<const Tables<double, KK>*>(m64.tabs[p])->op;               \
     if constexpr (sizeof(T) == 8) {                                                          \
       const SweepArgs<double> a = args[s];                                                   \
-      const auto& full = *static_cast<const FxFull<KK>*>(a.fx);                              \
+      const auto& full = *static_cast<const FxFull<KK>*>(m64.fx[p]);                         \
       double* sh = reinterpret_cast<double*>(smem_raw);                                      \
       if (kind == kPhSweep0)                                                                 \
         fxs_block<KK, 0, true>(full.band, full, op, a, blk, sh);                             \

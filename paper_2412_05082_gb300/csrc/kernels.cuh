@@ -107,7 +107,6 @@ struct SweepArgs {
   int64_t stride;  // n^axis
   double scale;
   int mode;
-  const void* fx;  // FP64: the fixed-point tables FxFull<K> (device)
 };
 
 // window w[j] = value at node c K - 2K + j, j in [LO, HI), zero outside 1..n;
