@@ -30,7 +30,7 @@ struct HostTables {
   FfTab<K>* ff = nullptr;
   FfTab<K>* dev_ff = nullptr;
   // FP64 tables only: the fixed-point tables (fx.cuh), the interior ones on the
-  // host (a kernel parameter), the others and D in device memory
+  // host (a kernel parameter), the others in device memory with D behind them
   FxCanon<K>* fx = nullptr;
   FxBand<K> band;
   FxFull<K>* dev_fx = nullptr;
@@ -44,36 +44,45 @@ static void free_host_tables(HostTables<T, K>* h) {
   cudaFree(h->dev);
   cudaFree(h->dev_ff);
   cudaFree(h->dev_fx);
-  cudaFree(h->dev_fxd);
   delete h->ff;
   delete h->fx;
   delete h;
 }
 
-// c 2^f as limbs of L bits
-static inline int2 fx_host(long double c, int f, int L) {
-  const long long v = std::llrint(std::ldexp(c, f));
+// limbs of L bits of an integer
+static inline int2 fx_host(long long v, int L) {
   const long long hi = (v + (1ll << (L - 1))) >> L;
   return make_int2((int)hi, (int)(v - hi * (1ll << L)));
 }
 
-// A row c 2^f as band limbs whose sum is rounded too: entries are rounded to
-// nearest, and then as many of those rounded furthest the other way as bring the
-// sum within half a unit.  The sum's error is what a smooth vector sees.
+// a / b 2^f rounded to nearest, as limbs: the quotient as a sum of two doubles (long
+// double is emulated in software on some hosts, and made this the larger part of a
+// context's creation)
+static inline int2 fx_host_quotient(double a, double b, int f, int L) {
+  const double hi = a / b, lo = std::fma(-hi, b, a) / b;
+  const double v = std::ldexp(hi, f), w = std::rint(v);
+  return fx_host((long long)w + std::llrint((v - w) + std::ldexp(lo, f)), L);
+}
+
+// A row c 2^f (c times a power of two: exact in FP64) as band limbs whose sum is
+// rounded too: entries are rounded to nearest, and then as many of those rounded
+// furthest the other way as bring the sum within half a unit.  The sum's error is
+// what a smooth vector sees.
 static inline void fx_host_row(const double* c, int n, double factor, int f, int2* out) {
-  long double v[4 * kMaxK + 1], d[4 * kMaxK + 1], err = 0;
+  double v[4 * kMaxK + 1], d[4 * kMaxK + 1], err = 0;
   int order[4 * kMaxK + 1];
+  const double scale = std::ldexp(factor, f);
   for (int t = 0; t < n; ++t) {
-    v[t] = std::ldexp((long double)c[t] * factor, f);
-    d[t] = v[t] - std::rint(v[t]);
+    const double x = c[t] * scale;
+    v[t] = std::rint(x);
+    d[t] = x - v[t];
     err += d[t];
     order[t] = t;
-    v[t] = std::rint(v[t]);
   }
   const int miss = (int)std::lround(err), step = miss < 0 ? -1 : 1;
   if (miss) std::sort(order, order + n, [&](int x, int y) { return step * d[x] > step * d[y]; });
   for (int i = 0; i < std::abs(miss) && i < n && d[order[i]] != 0; ++i) v[order[i]] += step;
-  for (int t = 0; t < n; ++t) out[t] = fx_host(v[t], 0, kFxBand);
+  for (int t = 0; t < n; ++t) out[t] = fx_host((long long)v[t], kFxBand);
 }
 
 // smallest e with v < 2^e, v a little enlarged: a coefficient's high limb has to
@@ -141,6 +150,8 @@ static FxScales fx_scales(const OpTab<double, K>& op, const FdmTab<double, K>& f
   return s;
 }
 
+// The sweeps' tables (every row at its own scale) and, in 2D, those of the patch
+// smoother, which is the fixed-point form only there.
 template <int K>
 static bool make_fx(HostTables<double, K>* h, const std::vector<double>& dinv, int md, int slots,
                     int d) {
@@ -149,42 +160,12 @@ static bool make_fx(HostTables<double, K>* h, const std::vector<double>& dinv, i
   const FdmTab<double, K>& fdm = h->t.fdm;
   const double(*tab[3])[BW] = {op.M, op.L, op.B};
   h->fx = new (std::nothrow) FxCanon<K>();
-  auto* full = new (std::nothrow) FxFull<K>();
-  // the division, for the 2D patch smoother's combinations
-  std::vector<int2> D(d == 2 ? dinv.size() : 1);
-  if (!h->fx || !full) {
-    delete full;
-    return false;
-  }
-  // interior: canonical rows 0..K-1, patch type 0
-  FxScales s = fx_scales<K>(op, fdm, K, 1);
-  int2* cx[3] = {h->fx->xM, h->fx->xL, h->fx->xB};
-  int2* cy[3] = {h->fx->yM, h->fx->yL, h->fx->yB};
-  int2 row[BW];
-  for (int o = 0; o < 3; ++o)
-    for (int q = 0; q < K; ++q) {
-      const int lo = band_lo(o, q, K), n = band_hi(o, q, K) - lo + 1;
-      fx_host_row(&tab[o][q][lo + 2 * K], n, 1.0, s.fx[o], row);
-      std::copy(row, row + n, cx[o] + FxIdx<K>::at(o, q, lo));
-      fx_host_row(&tab[o][q][lo + 2 * K], n, s.wy[o], s.gy, row);
-      std::copy(row, row + n, cy[o] + FxIdx<K>::at(o, q, lo));
-    }
-  auto fwd = [&](int ty, int j, int c) {
-    return fx_host((long double)fdm.S[ty][j][c] / s.cf, 2 * kFxLine - fx_col_exp(fdm.lam[ty][c]),
-                   kFxLine);
-  };
-  auto bwd = [&](int ty, int j, int c) {
-    return fx_host((long double)fdm.S[ty][j][c] / s.cb, 2 * kFxLine, kFxLine);
-  };
-  for (int j = 0; j < K; ++j)
-    for (int c = 0; c < M; ++c) {
-      h->fx->Sf[j][c] = fwd(0, j, c);
-      h->fx->Sb[j][c] = bwd(0, j, c);
-    }
-  h->fx->eax = -s.gy;
-  h->fx->corr = std::pow(s.cf * s.cb, d);
-  full->canon = *h->fx;
-  // sweeps: every row at its own scale
+  // FxFull<K> and, behind it, the division of the patch smoother's combinations
+  const size_t nD = d == 2 ? dinv.size() : 0, bytes = sizeof(FxFull<K>) + nD * sizeof(int2);
+  std::vector<unsigned char> buf(bytes);
+  if (!h->fx) return false;
+  auto* full = new (buf.data()) FxFull<K>();
+  int2* D = reinterpret_cast<int2*>(buf.data() + sizeof(FxFull<K>));
   int2* bx[3] = {h->band.M, h->band.L, h->band.B};
   float* ba[3] = {h->band.aM, h->band.aL, h->band.aB};
   for (int o = 0; o < 3; ++o)
@@ -196,50 +177,74 @@ static bool make_fx(HostTables<double, K>* h, const std::vector<double>& dinv, i
       fx_host_row(tab[o][c], BW, 1.0, f, full->s[o][c]);
       if (c >= K) continue;
       h->band.f[o][c] = f;
+      const double scale = std::ldexp(1.0, f - kFxCoef);
       for (int t = band_lo(o, c, K); t <= band_hi(o, c, K); ++t) {
         bx[o][FxIdx<K>::at(o, c, t)] = full->s[o][c][t + 2 * K];
-        ba[o][FxIdx<K>::at(o, c, t)] =
-            (float)std::ldexp(std::fabs(tab[o][c][t + 2 * K]), f - kFxCoef);
+        ba[o][FxIdx<K>::at(o, c, t)] = (float)(std::fabs(tab[o][c][t + 2 * K]) * scale);
       }
     }
   full->band = h->band;
-  // every class and type
-  s = fx_scales<K>(op, fdm, NC, 4);
-  for (int o = 0; o < 3; ++o)
-    for (int c = 0; c < NC; ++c) {
-      fx_host_row(tab[o][c], BW, 1.0, s.fx[o], full->x[o][c]);
-      fx_host_row(tab[o][c], BW, s.wy[o], s.gy, full->y[o][c]);
-    }
-  for (int ty = 0; ty < 4; ++ty)
-    for (int j = 0; j < M; ++j)
-      for (int c = 0; c < M; ++c) {
-        full->Sf[ty][j][c] = fwd(ty, j, c);
-        full->Sb[ty][j][c] = bwd(ty, j, c);
+  if (d == 2) {
+    // interior: canonical rows 0..K-1, patch type 0
+    FxScales s = fx_scales<K>(op, fdm, K, 1);
+    int2* cx[3] = {h->fx->xM, h->fx->xL, h->fx->xB};
+    int2* cy[3] = {h->fx->yM, h->fx->yL, h->fx->yB};
+    for (int o = 0; o < 3; ++o)
+      for (int q = 0; q < K; ++q) {
+        const int lo = band_lo(o, q, K), n = band_hi(o, q, K) - lo + 1, at = FxIdx<K>::at(o, q, lo);
+        fx_host_row(&tab[o][q][lo + 2 * K], n, 1.0, s.fx[o], cx[o] + at);
+        fx_host_row(&tab[o][q][lo + 2 * K], n, s.wy[o], s.gy, cy[o] + at);
       }
-  full->eax = -s.gy;
-  full->corr = std::pow(s.cf * s.cb, d);
-  std::vector<double> ds(md);  // the division, with the column scales taken back
-  for (int slot = 0; d == 2 && slot < slots; ++slot) {
-    double top = 0.0;
-    for (int l = 0; l < md; ++l) {
-      int e = 0, ll = l, ss = slot;
-      for (int a = 0; a < d; ++a, ll /= M, ss /= 4) e += fx_col_exp(fdm.lam[ss % 4][ll % M]);
-      ds[l] = std::ldexp(dinv[(size_t)slot * md + l], e);
-      top = std::max(top, std::fabs(ds[l]));
+    int ce[4][M];  // exponents of the forward lines' columns
+    for (int ty = 0; ty < 4; ++ty)
+      for (int c = 0; c < M; ++c) ce[ty][c] = fx_col_exp(fdm.lam[ty][c]);
+    auto fwd = [&](int ty, int j, int c) {
+      return fx_host_quotient(fdm.S[ty][j][c], s.cf, 2 * kFxLine - ce[ty][c], kFxLine);
+    };
+    auto bwd = [&](int ty, int j, int c) {
+      return fx_host_quotient(fdm.S[ty][j][c], s.cb, 2 * kFxLine, kFxLine);
+    };
+    for (int j = 0; j < K; ++j)
+      for (int c = 0; c < M; ++c) {
+        h->fx->Sf[j][c] = fwd(0, j, c);
+        h->fx->Sb[j][c] = bwd(0, j, c);
+      }
+    h->fx->eax = -s.gy;
+    h->fx->corr = std::pow(s.cf * s.cb, d);
+    full->canon = *h->fx;
+    // every class and type
+    s = fx_scales<K>(op, fdm, NC, 4);
+    for (int o = 0; o < 3; ++o)
+      for (int c = 0; c < NC; ++c) {
+        fx_host_row(tab[o][c], BW, 1.0, s.fx[o], full->x[o][c]);
+        fx_host_row(tab[o][c], BW, s.wy[o], s.gy, full->y[o][c]);
+      }
+    for (int ty = 0; ty < 4; ++ty)
+      for (int j = 0; j < M; ++j)
+        for (int c = 0; c < M; ++c) {
+          full->Sf[ty][j][c] = fwd(ty, j, c);
+          full->Sb[ty][j][c] = bwd(ty, j, c);
+        }
+    full->eax = -s.gy;
+    full->corr = std::pow(s.cf * s.cb, d);
+    double ds[M * M];  // the division, with the column scales taken back
+    for (int slot = 0; slot < slots; ++slot) {
+      const int *e0 = ce[slot % 4], *e1 = ce[slot / 4];
+      double top = 0.0;
+      for (int l = 0; l < md; ++l) {
+        ds[l] = std::ldexp(dinv[(size_t)slot * md + l], e0[l % M] + e1[l / M]);
+        top = std::max(top, std::fabs(ds[l]));
+      }
+      full->cD[slot] = top * (1.0 + 1e-9);
+      for (int l = 0; l < md; ++l)
+        D[(size_t)slot * md + l] = fx_host_quotient(ds[l], full->cD[slot], 2 * kFxLine, kFxLine);
     }
-    full->cD[slot] = top * (1.0 + 1e-9);
-    const long double inv = 1.0L / full->cD[slot];
-    for (int l = 0; l < md; ++l)
-      D[(size_t)slot * md + l] = fx_host(ds[l] * inv, 2 * kFxLine, kFxLine);
   }
-  const bool ok =
-      cudaMalloc(&h->dev_fx, sizeof(FxFull<K>)) == cudaSuccess &&
-      cudaMemcpy(h->dev_fx, full, sizeof(FxFull<K>), cudaMemcpyHostToDevice) == cudaSuccess &&
-      cudaMalloc(&h->dev_fxd, D.size() * sizeof(int2)) == cudaSuccess &&
-      cudaMemcpy(h->dev_fxd, D.data(), D.size() * sizeof(int2), cudaMemcpyHostToDevice) ==
-          cudaSuccess;
-  delete full;
-  return ok;
+  if (cudaMalloc(&h->dev_fx, bytes) != cudaSuccess ||
+      cudaMemcpy(h->dev_fx, buf.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess)
+    return false;
+  h->dev_fxd = reinterpret_cast<int2*>(h->dev_fx + 1);
+  return true;
 }
 
 template <typename T, int K>
