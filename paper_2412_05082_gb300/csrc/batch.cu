@@ -166,8 +166,10 @@ struct MvsOp {
   DevArray<MvsArgs<T>> args;
   DevArray<int> pid;
   DevArray<Tile> tiles;
-  DevArray<MvsArgs<T>> pargs;  // FP64: those of the persistent kernel
-  DevArray<Tile> ptiles;
+  // FP64: those of the persistent kernel, behind the others
+  const MvsArgs<T>* pargs = nullptr;
+  const Tile* ptiles = nullptr;
+  int nptiles = 0;
   size_t smem = 0;            // shared memory of a launch
   size_t psmem = 0;           // and of the persistent kernel's tiles
   int k = 0;                  // the degree of every problem of the op
@@ -629,13 +631,17 @@ bh_status build_vdepth(bh_batch* b, int t, VDepth<T>& V, Depth& D) {
       const int col = std::get<0>(key), k = std::get<1>(key);
       V.mvs[col].emplace_back();
       MvsOp<T>& op = V.mvs[col].back();
+      const size_t na = G.args.size(), nt = G.tiles.size();
+      G.args.insert(G.args.end(), G.pargs.begin(), G.pargs.end());
+      G.tiles.insert(G.tiles.end(), G.ptiles.begin(), G.ptiles.end());
       BCKS(upload(b, G.args, op.args));
       BCKS(upload(b, G.pid, op.pid));
       BCKS(upload(b, G.tiles, op.tiles));
-      if (sizeof(T) == 8) {
-        BCKS(upload(b, G.pargs, op.pargs));
-        BCKS(upload(b, G.ptiles, op.ptiles));
-      }
+      op.pargs = op.args.d + na;
+      op.ptiles = op.tiles.d + nt;
+      op.nptiles = op.tiles.n - (int)nt;
+      op.args.n = (int)na;
+      op.tiles.n = (int)nt;
       op.smem = smem_k[k];
       op.psmem = psmem_k[k];
       op.k = k;
@@ -1070,12 +1076,11 @@ struct PhaseBuilder {
         P.kind = kPhMvs;
       }
       MvsGroup& G = P.groups[P.ngroups++];
-      G.args = sizeof(T) == 8 ? op.pargs.d : op.args.d;
+      G.args = sizeof(T) == 8 ? op.pargs : op.args.d;
       G.pid = op.pid.d;
-      const DevArray<Tile>& tiles = sizeof(T) == 8 ? op.ptiles : op.tiles;
-      G.tiles = tiles.d;
-      G.ntiles = tiles.n;
-      P.total += tiles.n;
+      G.tiles = sizeof(T) == 8 ? op.ptiles : op.tiles.d;
+      G.ntiles = sizeof(T) == 8 ? op.nptiles : op.tiles.n;
+      P.total += G.ntiles;
       smem = std::max(smem, op.psmem);
     }
     ph.push_back(P);
