@@ -523,19 +523,19 @@ __device__ __forceinline__ void fdm_bwd_canon(const FdmT& fdm, const T* src, int
   }
 }
 
-// all patches of the tile interior: same stages as mvs2_tile.  COEF_DIRECT:
-// the coefficients are read from `op` and `fdm` themselves at compile-time
-// offsets -- for tables that are kernel parameters, constant-bank operands of
-// the FMAs, with no load instruction (FP32: 32 instead of 46 registers at
-// k = 4); otherwise they are staged in shared memory first (FP64 kernels,
-// whose constant operands the compiler hoists into 104-152 registers, and
-// tables in device memory).
+// all patches of the tile interior (FP32; FP64: fx2_tile of mvs_fx.cuh): same
+// stages as mvs2_tile.  COEF_DIRECT: the coefficients are read from `op` and `fdm`
+// themselves at compile-time offsets -- for tables that are kernel parameters,
+// constant-bank operands of the FMAs, with no load instruction (32 instead of 46
+// registers at k = 4); otherwise they are staged in shared memory first (tables in
+// device memory).
 template <typename T, int K, bool COEF_DIRECT = false, typename OpT = OpTab<T, K>,
           typename FdmT = FdmTab<T, K>>
 __device__ __forceinline__ void mvs2_tile_interior(const OpT& op, const FdmT& fdm,
                                                    const MvsArgs<T>& a, int first, int np,
                                                    unsigned char* smem_raw) {
   using C = Mvs2Cfg<T, K>;
+  static_assert(C::PREFETCH, "FP32");
   constexpr int M = C::M, W = C::W, WM = C::WM, MM = M * M;
   constexpr int WS = C::WS;
   const int pb = a.pb;
@@ -543,13 +543,11 @@ __device__ __forceinline__ void mvs2_tile_interior(const OpT& op, const FdmT& fd
   T* sTM = sX + pb * C::WIN;
   T* sTL = sTM + pb * W * M;
   T* sTB = sTL + pb * WM * M;
-  T* sBv = sTB + pb * WM * M;  // b on the patch nodes (PREFETCH)
-  // FP64: R and F over the window once the x-split has read it.  FP32: the
-  // window stays intact to the update, which reads x on the patch nodes from
-  // it; R takes the space after b, F that of T_M once the y-combination has
-  // read it
-  T* sR = C::PREFETCH ? sBv + pb * MM : sX;
-  T* sF = C::PREFETCH ? sTM : sR + pb * MM;
+  T* sBv = sTB + pb * WM * M;  // b on the patch nodes
+  // the window stays intact to the update, which reads x on the patch nodes from
+  // it; R takes the space after b, F that of T_M once the y-combination has read it
+  T* sR = sBv + pb * MM;
+  T* sF = sTM;
   __shared__ int sVi[32][2];
   // index in x of window node (0, 0) (negative for patches at v_a = 2), the
   // row offset of window row 0 in shared memory, and whether the window lies in
@@ -628,7 +626,7 @@ __device__ __forceinline__ void mvs2_tile_interior(const OpT& op, const FdmT& fd
       async_copy_or_zero(sX + e, a.x + (in ? (int64_t)(gy - 1) * n + (gx - 1) : 0), in);
     }
   }
-  if constexpr (C::PREFETCH) prefetch_patch_nodes<T, K, false>(a, np, sVi, sBv, nullptr);
+  prefetch_patch_nodes<T, K, false>(a, np, sVi, sBv, nullptr);
   async_copy_wait();
   __syncthreads();
   for (int e = threadIdx.x; e < 2 * np * W; e += blockDim.x) {
@@ -660,15 +658,12 @@ __device__ __forceinline__ void mvs2_tile_interior(const OpT& op, const FdmT& fd
     const T* cm = sTM + (p * W + K) * M + j;
     const T* cl = sTL + (p * WM) * M + j;
     const T* cb = sTB + (p * WM) * M + j;
-    const int g0 = K * (sVi[p][1] - 1);
-    const int gx = K * (sVi[p][0] - 1) + j + 1;
-    const T* bcol = C::PREFETCH ? sBv + p * MM + j : a.b + (int64_t)g0 * n + (gx - 1);
-    const int64_t bs = C::PREFETCH ? M : n;
+    const T* bcol = sBv + p * MM + j;
     T* rcol = sR + p * MM + j;
     if (half == 0)
-      ycombine_canon<T, K, 0>(op_s, cm, cl, cb, bcol, bs, asc, rcol);
+      ycombine_canon<T, K, 0>(op_s, cm, cl, cb, bcol, M, asc, rcol);
     else
-      ycombine_canon<T, K, 1>(op_s, cm, cl, cb, bcol, bs, asc, rcol);
+      ycombine_canon<T, K, 1>(op_s, cm, cl, cb, bcol, M, asc, rcol);
   }
   __syncthreads();
   // F = R S (rows)
@@ -719,13 +714,8 @@ __device__ __forceinline__ void mvs2_tile_interior(const OpT& op, const FdmT& fd
     const T* src = sF + p * MM + i * M;
     const int gy = K * (sVi[p][1] - 1) + i + 1, gx0 = K * (sVi[p][0] - 1) + 1;
     T* xrow = a.x + (int64_t)(gy - 1) * n + (gx0 - 1);
-    const T* xv = win_row(p, K + 1 + i) + K + 1;  // x on the row's patch nodes (PREFETCH)
-    auto put = [&](int j, T v) {
-      if constexpr (C::PREFETCH)
-        xrow[j] = xv[j] + ps * v;
-      else
-        xrow[j] += ps * v;
-    };
+    const T* xv = win_row(p, K + 1 + i) + K + 1;  // x on the row's patch nodes
+    auto put = [&](int j, T v) { xrow[j] = xv[j] + ps * v; };
     if (half == 0)
       fdm_bwd_canon<T, K, 0>(fdm_s, src, 1, put);
     else

@@ -425,9 +425,11 @@ void Ops<T>::free_tables(void* p, int k) {
 template <typename T, int K, int KIND>
 static cudaError_t launch_sweep(const HostTables<T, K>& h, const SweepArgs<T>& a, cudaStream_t st) {
   const int block = 128;
-  // FP64 on the integer pipe, except Q2 with less than one block per SM: there
-  // the FP64 form's little code is faster (apply on 32^2, 64^2, 128^2 cells 13.1,
-  // 14.1, 17.1 us against 14.9, 14.9, 15.2)
+  // FP64 on the integer pipe, except Q2 with less than one block per SM (152): there
+  // the FP64 form's little code is faster (apply on 8^3 and 16^3 cells 23.1 and 24.4
+  // us against 29.8 and 29.6; on 256^2 and 32^3, above the line, 31.7 and 56.2 against
+  // 27.7 and 51.6).  From Q3 on the smallest levels are even (2D Q3 16^2 18.4 against
+  // 17.0, 3D Q3 8^3 33.8 and 33.6) and the others faster (2D Q7 16^2 49.5 -> 37.7).
   bool fx = false;
   if constexpr (sizeof(T) == 8) {
     fx = K > 2 || split_blocks(a.lines, a.N) >= 152;
