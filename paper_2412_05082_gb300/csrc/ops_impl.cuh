@@ -425,14 +425,16 @@ void Ops<T>::free_tables(void* p, int k) {
 template <typename T, int K, int KIND>
 static cudaError_t launch_sweep(const HostTables<T, K>& h, const SweepArgs<T>& a, cudaStream_t st) {
   const int block = 128;
-  // FP64 on the integer pipe, except Q2 with less than one block per SM (152): there
-  // the FP64 form's little code is faster (apply on 8^3 and 16^3 cells 23.1 and 24.4
-  // us against 29.8 and 29.6; on 256^2 and 32^3, above the line, 31.7 and 56.2 against
-  // 27.7 and 51.6).  From Q3 on the smallest levels are even (2D Q3 16^2 18.4 against
-  // 17.0, 3D Q3 8^3 33.8 and 33.6) and the others faster (2D Q7 16^2 49.5 -> 37.7).
+  // FP64 on the integer pipe from one block per SM (152) on: apply of Q2 on 256^2 and
+  // 32^3 cells 31.7 and 56.2 -> 27.7 and 51.6 us, Q3 on 16^3 41.7 -> 31.6, Q7 on 8^3
+  // 124 -> 69.  Below, the FP64 form's little code is faster at Q2 (8^3 and 16^3 23.1
+  // and 24.4 against 29.8 and 29.6), even at Q3 and Q4, and slower from Q5 on on uniform
+  // values only (2D Q7 16^2 49.5 against 37.7): where rows are formed again, a launch of
+  // few blocks waits for them (a step with the exact solver on smoothed data, Q7 on
+  // 32^2, 1153 against 1250 to 1460, Q4 on 64^2 444 against 518).
   bool fx = false;
   if constexpr (sizeof(T) == 8) {
-    fx = K > 2 || split_blocks(a.lines, a.N) >= 152;
+    fx = split_blocks(a.lines, a.N) >= 152;
     if (fx)
       fxs_sweep_kernel<K, KIND><<<(unsigned)split_blocks(a.lines, a.N), block, 0, st>>>(
           h.band, h.dev_fx, h.dev, a);
