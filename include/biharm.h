@@ -314,12 +314,11 @@ bh_status bh_batch_vcycle_time(bh_batch* batch, int reps, double* ms);
  * operations and coarse solves of all problems at one depth -- separated by a
  * grid barrier.  Every barrier wait is bounded (2 s of clock cycles); a wait
  * that runs out ends the kernel with a status word that the next call reading
- * it turns into BH_ETIMEOUT.  Results equal the graph's up to rounding: in FP64
- * every patch takes the form that the graph uses on levels with few patches
- * (other scales of the same fixed-point arithmetic on large levels); the FP32
- * V-cycle's interior patches above degree 4 take the unfolded fast
- * diagonalization, its FP64 defects the FP64 pipe.  Host only.  BH_EINVAL for a
- * BH_MIXED_FP32_RC batch (its compensated defect sweeps are graph nodes only). */
+ * it turns into BH_ETIMEOUT.  Results equal the graph's up to rounding (FP64: tiles
+ * of other sizes, which on large levels decide the form a patch near the boundary
+ * takes; FP32 V-cycle: the unfolded fast diagonalization above degree 4, its FP64
+ * defects on the FP64 pipe).  Host only.  BH_EINVAL for a BH_MIXED_FP32_RC batch
+ * (its compensated defect sweeps are graph nodes only). */
 bh_status bh_batch_set_persistent(bh_batch* batch, int on);
 
 /* Check of the persistent form's failure path: one persistent V-cycle whose

@@ -271,6 +271,7 @@ struct bh_batch {
   long long graph_kernels = 0;   // kernel nodes of the captured V-cycle graph
   // persistent form: the V-cycle's phases for one cooperative launch
   bool persistent = false;
+  PersCoef<double> pcoef{};
   Phase* d_phases = nullptr;
   int nphases = 0;
   size_t psmem = 0;              // dynamic shared memory of the persistent kernel
@@ -580,7 +581,7 @@ bh_status build_vdepth(bh_batch* b, int t, VDepth<T>& V, Depth& D) {
     const int k = b->k[p];
     const int pb = std::min(mvs_pb(b, k), mvs_pb_max_t<T>(k));
     smem_k[k] = mvs_smem<T>(k, pb);
-    psmem_k[k] = mvs_smem<T>(k, sizeof(T) == 8 ? std::min(pb, kPersistentTile) : pb);
+    psmem_k[k] = mvs_smem<T>(k, sizeof(T) == 8 ? std::min(pb, persistent_tile(k)) : pb);
     const DevTables dt = Ops<T>::device_tables(LvBuf<T>::tab(c), k);
     // one launch per class of problems whose interior tables agree byte for
     // byte (one penalty), the tables being the launch's parameter
@@ -615,9 +616,9 @@ bh_status build_vdepth(bh_batch* b, int t, VDepth<T>& V, Depth& D) {
       for (int f = (a.count - 1) / step * step; a.count > 0 && f >= 0; f -= step)
         G.tiles.push_back(Tile{s, f, std::min(step, a.count - f)});
       if (sizeof(T) == 8) {
-        a.pb = std::min(pb, kPersistentTile);
+        a.pb = std::min(pb, persistent_tile(k));
         G.pargs.push_back(a);
-        for (int f = 0, pt = std::min(step, kPersistentTile); f < a.count; f += pt)
+        for (int f = 0, pt = std::min(step, a.pb); f < a.count; f += pt)
           G.ptiles.push_back(Tile{s, f, std::min(pt, a.count - f)});
       }
     }
@@ -1065,6 +1066,29 @@ struct PhaseBuilder {
   void conv(const ConvOpList& op, int dir) {
     list(kPhConv, op.pid.n, op.total, op.v.d, op.prefix.d, op.pid.d, dir);
   }
+  // the kernel's parameter tables: the first class of every degree
+  PersCoef<double>* coef = nullptr;
+  const void* taken[kMaxK + 1] = {nullptr};
+  template <int K>
+  bool canon_k(const void* htab) {
+    auto* dst = const_cast<FxCanon<K>*>(&coef->template at<K>());
+    if (!taken[K]) {
+      taken[K] = htab;
+      std::memcpy(dst, htab, sizeof(*dst));
+    }
+    return std::memcmp(dst, htab, sizeof(*dst)) == 0;
+  }
+  bool canon(const MvsOp<T>& op) {
+    if (sizeof(T) != 8) return false;
+    switch (op.k) {
+      case 2: return canon_k<2>(op.htab);
+      case 3: return canon_k<3>(op.htab);
+      case 4: return canon_k<4>(op.htab);
+      case 5: return canon_k<5>(op.htab);
+      case 6: return canon_k<6>(op.htab);
+      default: return canon_k<7>(op.htab);
+    }
+  }
   void mvs(const std::vector<MvsOp<T>>& ops) {
     if (ops.empty()) return;
     Phase P{};
@@ -1080,6 +1104,7 @@ struct PhaseBuilder {
       G.pid = op.pid.d;
       G.tiles = sizeof(T) == 8 ? op.ptiles : op.tiles.d;
       G.ntiles = sizeof(T) == 8 ? op.nptiles : op.tiles.n;
+      G.canon = canon(op);
       P.total += G.ntiles;
       smem = std::max(smem, op.psmem);
     }
@@ -1094,6 +1119,7 @@ template <typename T>
 bh_status build_phases(bh_batch* b, const TopOps& top) {
   std::vector<Phase> ph;
   PhaseBuilder<T> B{ph};
+  B.coef = &b->pcoef;
   const int T_ = (int)b->depth.size();
   if (b->mixed) {
     B.zero(vdepth_top<T>(top));
@@ -1175,7 +1201,9 @@ bh_status launch_persistent(bh_batch* b, unsigned extra, long long budget) {
   unsigned* bar = b->d_bar;
   unsigned expected = (unsigned)b->pgrid + extra;
   int* status = reinterpret_cast<int*>(b->d_bar + 2);
-  void* args[] = {&m64, &mT, &phases, &nph, &bar, &expected, &status, &budget};
+  PersCoef<float> none{};
+  void* coef = b->mixed ? (void*)&none : (void*)&b->pcoef;
+  void* args[] = {&m64, &mT, &phases, &nph, &bar, &expected, &status, &budget, coef};
   const void* kernel = b->mixed ? vcycle_persistent_kernel_for<float>()
                                 : vcycle_persistent_kernel_for<double>();
   BCK(cudaLaunchCooperativeKernel(kernel, dim3(b->pgrid), dim3(256), args, b->psmem, b->st));

@@ -249,6 +249,7 @@ struct MvsGroup {  // the tiles of one degree in an MVS phase
   const int* pid;
   const Tile* tiles;
   int ntiles;
+  int canon;          // FP64: the interior tables are the kernel's (PersCoef)
 };
 
 struct Phase {
@@ -301,9 +302,51 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned* gen, uns
   return ok != 0;
 }
 
-// Patches per tile of the persistent kernel in FP64 at most (1, 2, 4: 93, 72, 61 ms
-// for a V-cycle of 64 problems; 8: 92, its shared memory leaves one block per SM).
-constexpr int kPersistentTile = 4;
+// Interior tables of every degree, the FP64 persistent kernel's parameter (constant-
+// bank operands, as in the graph's kernels); problems of another penalty take the
+// latency form
+template <typename T>
+struct PersCoef {
+  int unused;
+};
+template <>
+struct PersCoef<double> {
+  FxCanon<2> c2;
+  FxCanon<3> c3;
+  FxCanon<4> c4;
+  FxCanon<5> c5;
+  FxCanon<6> c6;
+  FxCanon<7> c7;
+  template <int K>
+  __host__ __device__ __forceinline__ const FxCanon<K>& at() const {
+    if constexpr (K == 2) return c2;
+    else if constexpr (K == 3) return c3;
+    else if constexpr (K == 4) return c4;
+    else if constexpr (K == 5) return c5;
+    else if constexpr (K == 6) return c6;
+    else return c7;
+  }
+};
+
+// Patches per tile of the FP64 persistent kernel at most: what fits twice on an SM
+// beside the static shared memory of all degrees' tile code (at 84 KB one block fits, and
+// the V-cycle of 64 problems takes 68 ms instead of 46)
+constexpr int kPersistentSmem = 60 * 1024;
+template <int K>
+constexpr int persistent_tile() {
+  constexpr int fit = (kPersistentSmem / 8 - Fx2Cfg<K>::MM) / Fx2Cfg<K>::PER;
+  return fit < 1 ? 1 : (fit > 32 ? 32 : fit);
+}
+inline int persistent_tile(int k) {
+  switch (k) {
+    case 2: return persistent_tile<2>();
+    case 3: return persistent_tile<3>();
+    case 4: return persistent_tile<4>();
+    case 5: return persistent_tile<5>();
+    case 6: return persistent_tile<6>();
+    default: return persistent_tile<7>();
+  }
+}
 
 // thread `t` of a 32-line x 4-cell tile (block blk) of a 2D sweep, with plain loads:
 // the inputs were written by an earlier phase
@@ -326,15 +369,16 @@ __device__ __forceinline__ void sweep_tile_coherent(const OpTab<double, K>& op,
   }
 }
 
-// One kernel holds the code of every degree (128 registers, spills), so the tiles
-// take the form of the fixed-point smoother with the least of it, the latency form,
-// and the defects of the FP32 V-cycle the FP64 sweeps.  A V-cycle of 64 problems: FP64
-// with the graph's unrolled tiles 74 ms, on the FP64 pipe 68, this way 61 (the graph
-// 38); FP32 with FP64 defects 27 with fixed-point sweeps, 24 this way.
+// One kernel holds the code of every degree (128 registers, spills).  V-cycle of 64
+// problems with tuned tiles (the graph 34 ms): on the FP64 pipe 47 ms, fixed point with
+// the tables in memory and one block per SM 74, the latency form for all tiles 59, this
+// way 46.  The defects of the FP32 V-cycle take the FP64 sweeps: 24 ms, with fixed-point
+// sweeps 27.
 template <typename T>
 __global__ void __launch_bounds__(256, 2) vcycle_persistent_kernel(
     Meta m64, Meta mT, const Phase* __restrict__ phases, int nphases, unsigned* bar,
-    unsigned expected, int* status, long long budget) {
+    unsigned expected, int* status, long long budget,
+    const __grid_constant__ PersCoef<T> coef) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t gthreads = (int64_t)gridDim.x * blockDim.x;
@@ -440,7 +484,8 @@ __global__ void __launch_bounds__(256, 2) vcycle_persistent_kernel(
   {                                                                                           \
     const auto* tb = static_cast<const Tables<T, KK>*>(mT.tabs[p]);                           \
     if constexpr (sizeof(T) == 8)                                                             \
-      fx2_small_tile<KK>(tb, args[tile.s], tile.first, tile.count, smem_raw);                 \
+      fx2_any_tile<KK>(coef.template at<KK>(), tb, args[tile.s], tile.first, tile.count,      \
+                       !G.canon || args[tile.s].count <= kFx2SmallCount, smem_raw);           \
     else if (KK <= kBatchInteriorMaxK && mvs2_tile_is_interior(args[tile.s], tile.first, tile.count)) \
       mvs2_tile_interior<T, KK>(tb->op, tb->fdm, args[tile.s], tile.first, tile.count, smem_raw); \
     else                                                                                      \
