@@ -811,10 +811,11 @@ def main():
         "bound": "alu", "achieved": achieved, "peak": FX_PEAK_TFLOPS, "unit": "TFLOP/s",
         "frac": achieved / FX_PEAK_TFLOPS,
         # dram__bytes_read.sum + dram__bytes_write.sum of one launch of this kernel in this
-        # configuration, from one ncu capture (63.1 MB + 2.4 MB)
-        "traffic": 65.5e6, "traffic_unit": "bytes per launch",
+        # configuration, from one ncu capture (63.0 MB + 3.0 MB)
+        "traffic": 66.0e6, "traffic_unit": "bytes per launch",
         "peak_source": "integer pipe: 152 SMs x 63 IMAD.WIDE/clk (measured) x 2070 MHz, three per "
-                       "FP64 FMA; the kernel is bound by instruction issue, of which these are a third",
+                       "FP64 FMA; the kernel issues on 43 % of its cycles, a third of it these, and waits "
+                       "on barriers and fixed latencies at 22 warps per SM",
         "fp64_pipe_peak_tflops": FP64_PEAK_TFLOPS, "frac_of_fp64_pipe": achieved / FP64_PEAK_TFLOPS,
         "measured_peak_tflops": probe,
         "measured_peak_source": "the library's FP64 FMA probe on this GPU (bh_fp64_fma_rate: "
@@ -822,7 +823,7 @@ def main():
         "frac_of_measured_peak": achieved / probe,
         "hbm_roofline": "not the bound: integer-pipe machine balance / measured HBM copy bandwidth "
                         "= %.2f flop/B, while this kernel does about %.0f flop per DRAM byte"
-                        % (FX_PEAK_TFLOPS * 1e12 / (HBM_GBS * 1e9), flops_launch / 65.5e6),
+                        % (FX_PEAK_TFLOPS * 1e12 / (HBM_GBS * 1e9), flops_launch / 66.0e6),
         "fma_per_patch": mvs2_fma_per_patch(k), "patches_per_launch": patches / 8,
         "launch_ms": t_step / 8 * 1e3,
     }
